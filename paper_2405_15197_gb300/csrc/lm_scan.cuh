@@ -171,7 +171,8 @@ static __global__ void __launch_bounds__(SCAN_THREADS) k_scans_apply(ScanJobs J,
     v[q] = i < n ? (int64_t)J.in[j][i * J.stride[j]] : 0;
     s += v[q];
   }
-  int64_t off = block_excl_scan(s, wt, &tot) + (sums ? sums[j * nb + blockIdx.x] : 0);
+  // (the first block's offset is zero; an empty array has no block sum at all)
+  int64_t off = block_excl_scan(s, wt, &tot) + (sums && blockIdx.x > 0 ? sums[j * nb + blockIdx.x] : 0);
 #pragma unroll
   for (int q = 0; q < SCAN_ITEMS; q++) {
     const int64_t i = base + q;

@@ -1,7 +1,8 @@
 """Calls at the ends of the accepted range:
 
 * objective and adjoint at resolutions where the shared memory holds two
-  8-lane stitching tiles per block, which are half a warp.
+  8-lane stitching tiles per block, which are half a warp;
+* lattices without struts whose node arrays span several scan tiles.
 """
 import numpy as np
 import pytest
@@ -34,5 +35,28 @@ def test_objective_at_fine_resolution(dtype, k, adjoint):
     if adjoint:
         _, _, a, v = mm.backward(k, 1.0, 0.5)
         assert (a, v) == pytest.approx((area, vol), rel=tol)
+    assert liblm.lm_last_error(mm.h) == 0
+    mm.close()
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("nodes", [4096, 4097, 5000, 10000])
+def test_nodes_without_struts(nodes, dtype):
+    """An empty meta-mesh: the scan over the strut ends is of an empty array
+    beside arrays of several tiles (4,096 elements).  The memory is that of a
+    larger build freed before, so what is not written shows."""
+    dirty = liblm.MetaMesh(*P.to_device(P.lattice_as(L.octet(8), dtype), dtype))
+    dirty.tri_count(8)
+    dirty.close()
+    t = torch.float32 if dtype == np.float32 else torch.float64
+    mm = liblm.MetaMesh(torch.rand((nodes, 3), dtype=t, device="cuda"),
+                        torch.zeros((0, 2), dtype=torch.int32, device="cuda"),
+                        torch.zeros((0, 2), dtype=t, device="cuda"))
+    assert mm.counts()[:5] == [0, 0, 0, 0, 0]
+    g = mm.download()
+    assert len(g["loop_ent"]) == 0 and np.array_equal(g["end_off"], [0])
+    for key in ("row_ptr", "vtx_off", "arc_off", "hole_off_n"):
+        assert np.array_equal(g[key], np.zeros(nodes + 1)), key
+    assert mm.tri_count(8) == 0 and mm.objective(8) == (0.0, 0.0)
     assert liblm.lm_last_error(mm.h) == 0
     mm.close()
