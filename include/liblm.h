@@ -38,7 +38,10 @@ typedef enum {
                                  or NaN, coordinate NaN, k out of [1, 4096] */
   LM_ERR_RADIUS_MISMATCH = 2, /* two strut ends at one node carry radii that
                                  differ by more than 1e-12 relative */
-  LM_ERR_DEGENERATE = 3,      /* a strut with |R_a - R_b| >= its length */
+  LM_ERR_DEGENERATE = 3,      /* a strut with |R_a - R_b| >= its length, to
+                                 the rounding of the lattice's type; or its
+                                 length or a radius, squared, outside that
+                                 type's normal numbers */
   LM_ERR_CAPACITY = 4,        /* an output or per-node work buffer too small */
   LM_ERR_OOM = 5,             /* device allocation failed */
   LM_ERR_CUDA = 6,            /* a CUDA runtime call failed */

@@ -212,7 +212,19 @@ __global__ void k_strut_taper(const T* xyz, const int32_t* ends, const T* node_R
     double dx = (double)xyz[3 * b] - (double)xyz[3 * a], dy = (double)xyz[3 * b + 1] - (double)xyz[3 * a + 1],
            dz = (double)xyz[3 * b + 2] - (double)xyz[3 * a + 2];
     double L = sqrt(dx * dx + dy * dy + dz * dz);
-    if (!(fabs((double)node_R[a] - (double)node_R[b]) < L)) set_err(err, LM_ERR_DEGENERATE);
+    bool ok = fabs((double)node_R[a] - (double)node_R[b]) < L;
+    // The same in the lattice's type, in which the kernels form the strut's
+    // direction and cone (make_end): where the length or a radius squared
+    // leaves the normal numbers, or the cosine of the half-angle is down to
+    // the rounding of 1 - s^2, they would be infinite or NaN.
+    constexpr T least = sizeof(T) == 4 ? T(1.17549435e-38) : T(2.2250738585072014e-308);
+    constexpr T most = sizeof(T) == 4 ? T(3.40282347e38) : T(1.7976931348623157e308);
+    constexpr T ulp = sizeof(T) == 4 ? T(1.1920929e-7) : T(2.220446049250313e-16);
+    const T tx = xyz[3 * b] - xyz[3 * a], ty = xyz[3 * b + 1] - xyz[3 * a + 1], tz = xyz[3 * b + 2] - xyz[3 * a + 2];
+    const T L2 = tx * tx + ty * ty + tz * tz, Ra = node_R[a], Rb = node_R[b];
+    const T s = (Ra - Rb) * (T(1) / sqrt(L2));
+    ok = ok && L2 >= least && L2 <= most && Ra * Ra <= most && Rb * Rb <= most && T(1) - s * s >= T(4) * ulp;
+    if (!ok) set_err(err, LM_ERR_DEGENERATE);
   }
 }
 

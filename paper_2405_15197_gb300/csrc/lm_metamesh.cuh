@@ -735,7 +735,8 @@ __device__ __forceinline__ void node_loops(WarpSmem<T, C>& S, const MMArgs<T>& A
       // strut's length: degenerate nodes) amplifies its FP32 position
       // error: the loop is ordered with FP64 angles
       if (!IS64 && T(256) * (zx * zx + zy * zy) < dot(z, z) + R * R) uncm |= 1ull << i;
-      S.le_dphi[e] = norm_angle(a);
+      // (an angle that is no number sorts last: every entry has a place)
+      S.le_dphi[e] = a == a ? norm_angle(a) : T(INFINITY);
       S.le_v[e] = (uint8_t)v;
       S.le_ang[e] = S.le_dphi[e];
     }
@@ -753,7 +754,7 @@ __device__ __forceinline__ void node_loops(WarpSmem<T, C>& S, const MMArgs<T>& A
         p += (x < a || (x == a && q < e)) ? 1 : 0;
       }
       S.le_v[p] = S.le_rev[e];
-      S.le_ang[p] = a;
+      S.le_ang[p] = a < T(INFINITY) ? a : T(NAN);
     }
     __syncwarp();
     if constexpr (!IS64) {

@@ -2,7 +2,8 @@
 
 * objective and adjoint at resolutions where the shared memory holds two
   8-lane stitching tiles per block, which are half a warp;
-* lattices without struts whose node arrays span several scan tiles.
+* lattices without struts whose node arrays span several scan tiles;
+* struts whose length, radius or taper leaves the range of the lattice's type.
 """
 import numpy as np
 import pytest
@@ -59,4 +60,43 @@ def test_nodes_without_struts(nodes, dtype):
         assert np.array_equal(g[key], np.zeros(nodes + 1)), key
     assert mm.tri_count(8) == 0 and mm.objective(8) == (0.0, 0.0)
     assert liblm.lm_last_error(mm.h) == 0
+    mm.close()
+
+
+def one_strut(length, ra, rb):
+    return {"xyz": np.array([[0.0, 0.0, 0.0], [0.0, 0.0, length]]), "ends": np.array([[0, 1]], dtype=np.int32),
+            "radii": np.array([[ra, rb]]), "name": "one"}
+
+
+# Refused: squared length or radius below or above the type's normal numbers,
+# taper within the rounding of 1 - s^2 of the limit.
+@pytest.mark.parametrize("dtype,length,ra,rb", [
+    (np.float32, 1e-20, 1e-21, 1e-21), (np.float32, 1e-19, 1e-20, 1e-20), (np.float32, 3e19, 1.0, 1.0),
+    (np.float32, 1e10, 1e20, 1e20), (np.float32, 1.0, 1.5, 0.5 + 2.0 ** -24), (np.float32, 1.0, 0.5 + 2.0 ** -24, 1.5),
+    (np.float64, 1e-155, 1e-156, 1e-156), (np.float64, 1e155, 1.0, 1.0), (np.float64, 1e10, 1e155, 1e155),
+    (np.float64, 1.0, 1.5, 0.5 + 2.0 ** -53)])
+def test_struts_outside_the_range_of_the_type(dtype, length, ra, rb):
+    """Such a strut's direction or cone would be infinite or NaN in the
+    kernels, and with it angles that loops are ordered by."""
+    x, e, r = P.to_device(one_strut(length, ra, rb), dtype)
+    assert float(r[0, 0]) > 0 and abs(float(r[0, 0]) - float(r[0, 1])) < float(x[1, 2])
+    with pytest.raises(liblm.LmError) as ei:
+        liblm.MetaMesh(x, e, r)
+    assert ei.value.status == 3
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_struts_inside_the_range_of_the_type(dtype):
+    """Scaled by a power of two, a lattice keeps its meta-mesh; a steep taper
+    above the rounding is accepted."""
+    lat = P.lattice_as(L.bcc(2, jitter=0.05, radius_range=(0.05, 0.09)), dtype)
+    mm = liblm.MetaMesh(*P.to_device(lat, dtype))
+    want = mm.counts()
+    mm.close()
+    for s in (2.0 ** -50, 2.0 ** 50):
+        mm = liblm.MetaMesh(*P.to_device(dict(lat, xyz=lat["xyz"] * s, radii=lat["radii"] * s), dtype))
+        assert mm.counts() == want
+        mm.close()
+    mm = liblm.MetaMesh(*P.to_device(one_strut(1.0, 1.5, 0.5 + 1e-5), dtype))
+    assert mm.counts()[:4] == [2, 0, 2, 2]
     mm.close()
