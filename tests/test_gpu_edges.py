@@ -3,7 +3,8 @@
 * objective and adjoint at resolutions where the shared memory holds two
   8-lane stitching tiles per block, which are half a warp;
 * lattices without struts whose node arrays span several scan tiles;
-* struts whose length, radius or taper leaves the range of the lattice's type.
+* struts whose length, radius or taper leaves the range of the lattice's type;
+* an objective whose sums leave the range of FP32.
 """
 import numpy as np
 import pytest
@@ -100,3 +101,20 @@ def test_struts_inside_the_range_of_the_type(dtype):
     mm = liblm.MetaMesh(*P.to_device(one_strut(1.0, 1.5, 0.5 + 1e-5), dtype))
     assert mm.counts()[:4] == [2, 0, 2, 2]
     mm.close()
+
+
+def test_objective_sums_beyond_fp32():
+    """The sums are FP64: a lattice 1,024 cells from the origin, scaled by
+    2^42, has terms of the volume above 10^39.  Scaling by a power of two
+    changes no rounding, so the volume scales by 2^126; the order of the sums
+    is free (terms 100 times the total, 10^-14 each)."""
+    lat = P.lattice_as(L.bcc(2, radius=0.0625), np.float32)
+    got = []
+    for s in (1.0, 2.0 ** 42):
+        mm = liblm.MetaMesh(*P.to_device(dict(lat, xyz=(lat["xyz"] + 1024.0) * s, radii=lat["radii"] * s), np.float32))
+        mm.tri_count(8)
+        v = mm.objective(8)[1] / s ** 3
+        assert mm.backward(8, 0.0, 1.0)[3] / s ** 3 == pytest.approx(v, rel=1e-10)
+        got.append(v)
+        mm.close()
+    assert got[1] == pytest.approx(got[0], rel=1e-10)
