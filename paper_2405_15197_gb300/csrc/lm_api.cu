@@ -696,7 +696,18 @@ lm_status build_impl(lm_metamesh* mm, cudaStream_t st) {
   mm->max_loop_entries = (int)hb.stat[2];
   // FP64 fallback contexts of the triangulation kernels
   mm->scratch_warps = tri_scratch_warps(N, E);
-  LM_CK(mm_malloc(mm, (void**)&mm->scratch, node64_bytes() * (size_t)mm->scratch_warps, st));
+  {
+    const size_t bytes = node64_bytes() * (size_t)mm->scratch_warps;
+    cudaError_t se = mm_malloc(mm, (void**)&mm->scratch, bytes, st);
+    if (se == cudaErrorMemoryAllocation) {
+      // no room beside the arena and the temporaries, which nothing reads any
+      // more: their memory serves (the frees are in stream order)
+      (void)cudaGetLastError();
+      free_build_temps(mm, st);
+      se = mm_malloc(mm, (void**)&mm->scratch, bytes, st);
+    }
+    LM_CK(se);
+  }
   LM_CK(cudaStreamSynchronize(st));
   cudaEventElapsedTime(&mm->t_csr, ev[0], ev[1]);
   cudaEventElapsedTime(&mm->t_count, ev[1], ev[2]);

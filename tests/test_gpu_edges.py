@@ -4,7 +4,8 @@
   8-lane stitching tiles per block, which are half a warp;
 * lattices without struts whose node arrays span several scan tiles;
 * struts whose length, radius or taper leaves the range of the lattice's type;
-* an objective whose sums leave the range of FP32.
+* an objective whose sums leave the range of FP32;
+* a device with room for the build but not for the arena beside it.
 """
 import numpy as np
 import pytest
@@ -118,3 +119,37 @@ def test_objective_sums_beyond_fp32():
         got.append(v)
         mm.close()
     assert got[1] == pytest.approx(got[0], rel=1e-10)
+
+
+def test_build_where_the_arena_leaves_no_room():
+    """What fits without the arena fits with it: on a device filled up to 64
+    MB above the needs of a build without one, the default build (an arena of
+    about 140 MB) gives way, also after its outputs are allocated (the FP64
+    contexts come last, about 160 MB)."""
+    x, e, r = P.to_device(P.lattice_as(L.bcc(40, radius=0.05), np.float32), np.float32)
+    none = liblm.lm_options()
+    none.arena_bytes = -1
+    total = torch.cuda.mem_get_info()[1]
+    liblm.MetaMesh(x, e, r).close()  # every kernel is loaded
+    liblm.lm_pool_retain(0)
+    filler = None
+    try:
+        liblm.lm_pool_retain((1 << 64) - 1)
+        torch.cuda.empty_cache()
+        free0 = torch.cuda.mem_get_info()[0]
+        mm = liblm.MetaMesh(x, e, r, options=none)
+        need = free0 - torch.cuda.mem_get_info()[0]
+        want = mm.counts()
+        mm.close()
+        liblm.lm_pool_retain(0)
+        filler = torch.empty(torch.cuda.mem_get_info()[0] - need - (64 << 20), dtype=torch.uint8, device="cuda")
+        for opt in (none, None):
+            mm = liblm.MetaMesh(x, e, r, options=opt)
+            assert mm.counts() == want
+            assert mm.tri_count(8) > 0
+            mm.close()
+            liblm.lm_pool_retain(0)
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+        liblm.lm_pool_retain(total // 16)
