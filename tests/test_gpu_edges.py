@@ -42,6 +42,27 @@ def test_objective_at_fine_resolution(dtype, k, adjoint):
     mm.close()
 
 
+@pytest.mark.parametrize("dtype,k", [(np.float32, 1200), (np.float64, 650)])
+def test_adjoint_at_fine_resolution(dtype, k):
+    """Gradients where the adjoint takes 16-lane tiles, against central
+    differences of the oracle's frozen structure (bounds of test_gpu_adjoint)."""
+    lat = P.lattice_as(L.bcc(1, jitter=0.05, radius_range=(0.05, 0.09)), dtype)
+    o = oracle.Oracle(lat)
+    fz = oracle.Frozen(o, k)
+    d1, d2 = (np.stack(fz.fd(h, np.arange(o.N))) for h in (1e-4, 5e-5))
+    ref = (4.0 * d2 - d1) / 3.0
+    ref = 1.0 * ref[0] + 0.5 * ref[1]
+    mm = liblm.MetaMesh(*P.to_device(lat, dtype))
+    gx, gr, _, _ = mm.backward(k, 1.0, 0.5)
+    g = np.concatenate([gx.cpu().numpy(), gr.cpu().numpy()[:, None]], 1).astype(np.float64)
+    err = np.abs(g - ref)
+    if dtype == np.float32:
+        assert err.max() < 1e-3 * np.abs(ref).max()
+    else:
+        assert (err / np.maximum(np.abs(ref), 1e-3 * np.abs(ref).max())).max() < 1e-6
+    mm.close()
+
+
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])
 @pytest.mark.parametrize("nodes", [4096, 4097, 5000, 10000])
 def test_nodes_without_struts(nodes, dtype):
