@@ -423,7 +423,7 @@ def bench_gpu(args):
         "valence_histogram": {str(d): c for d, c in sorted(vhist.items())},
         "fp64_stability_steps": fp64,
         "metamesh_launch_shape": {"buckets": ["d<=16", "d<=32", "d<=64"],
-                                  "warps_per_block_nodes_per_pop": launch_shape, "autotuned": True,
+                                  "warps_of_every_four_nodes_per_pop": launch_shape, "autotuned": True,
                                   "nodes_computed_twice": twice},
         "roofline": roof,
         "rooflines": roofs,
@@ -524,7 +524,7 @@ def bench_irregular(torch, liblm, dev, stream, k=16, reps=3):
             "near_tangent_fraction": float(np.mean((flags & 1) != 0)),
             "meta_mesh_counts": counts[:6], "fp64_stability_steps": fb,
             "metamesh_launch_shape": {"buckets": ["d<=16", "d<=32", "d<=64"],
-                                      "warps_per_block_nodes_per_pop": shape, "autotuned": True},
+                                      "warps_of_every_four_nodes_per_pop": shape, "autotuned": True},
             "timing": f"median of {reps} (CUDA events)"}
 
 

@@ -326,7 +326,7 @@ lm_status lm_metamesh_backward(lm_metamesh* mm, int32_t k, double w_area, double
  * of a block that work on the bucket (the others' shared memory holds its
  * larger workspaces), out[2b+1] = nodes a warp takes per work-queue access.  With
  * lm_options.autotune these are the autotuner's choices (Section 4.3.3's
- * workload balancing, done by measurement); 0 for buckets without nodes.
+ * workload balancing, done by measurement).  A block has sixteen warps.
  * out[6] = nodes the emit pass computed a second time (those the count
  * pass's arena could not hold; every node when the build ran without an
  * arena), out[7] = 1 if the emit pass took only those nodes from the lists

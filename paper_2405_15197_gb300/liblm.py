@@ -394,7 +394,8 @@ class MetaMesh:
 
 
 def lm_metamesh_launch_shape(h):
-    """[(warps per block, nodes per queue access)] per valence bucket."""
+    """[(warps of every four of a block that work on it, nodes a warp takes per
+    queue access)] per valence bucket; a block has sixteen warps."""
     out = (ctypes.c_int32 * 8)()
     _ck(load().lm_metamesh_launch_shape(h, out), "lm_metamesh_launch_shape")
     return [(out[2 * b], out[2 * b + 1]) for b in range(3)]
