@@ -5,7 +5,8 @@
 * lattices without struts whose node arrays span several scan tiles;
 * struts whose length, radius or taper leaves the range of the lattice's type;
 * an objective whose sums leave the range of FP32;
-* a device with room for the build but not for the arena beside it.
+* a device with room for the build but not for the arena beside it;
+* memory that the pool keeps, and gives back on request.
 """
 import numpy as np
 import pytest
@@ -150,7 +151,6 @@ def test_build_where_the_arena_leaves_no_room():
     x, e, r = P.to_device(P.lattice_as(L.bcc(40, radius=0.05), np.float32), np.float32)
     none = liblm.lm_options()
     none.arena_bytes = -1
-    total = torch.cuda.mem_get_info()[1]
     liblm.MetaMesh(x, e, r).close()  # every kernel is loaded
     liblm.lm_pool_retain(0)
     filler = None
@@ -173,4 +173,20 @@ def test_build_where_the_arena_leaves_no_room():
     finally:
         del filler
         torch.cuda.empty_cache()
-        liblm.lm_pool_retain(total // 16)
+
+
+def test_pool_keeps_and_gives_back():
+    """A build of about 440 MB (BCC 40^3 with its arena) stays mapped after it
+    is freed, up to the limit; lm_pool_retain(0) returns it to the device."""
+    x, e, r = P.to_device(P.lattice_as(L.bcc(40, radius=0.05), np.float32), np.float32)
+    liblm.MetaMesh(x, e, r).close()  # every kernel is loaded
+    liblm.lm_pool_retain(0)
+    torch.cuda.synchronize()
+    free0, total = torch.cuda.mem_get_info()
+    liblm.lm_pool_retain(total // 16)
+    liblm.MetaMesh(x, e, r).close()
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] < free0 - (200 << 20)
+    liblm.lm_pool_retain(0)
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] > free0 - (64 << 20)
