@@ -107,3 +107,42 @@ def test_adjoint_accumulates_and_autograd():
     g2 = torch.ones((o.N,), device="cuda")
     liblm.lm_metamesh_backward(mm.h, K, 1.0, 0.0, g1.data_ptr(), g2.data_ptr())
     assert np.allclose(g1.cpu().numpy() - 1.0, ga[:, :3], rtol=0, atol=1e-3 * np.abs(ga).max())
+
+
+@pytest.mark.parametrize("name,k", [("jittered", 7), ("jittered", 32), ("octet", 16), ("octet", 9)])
+def test_fp32_adjoint_error(name, k):
+    """FP32 gradients against the FP64 lattice's in the 2-norm: 6e-8 to 4e-7
+    measured on such lattices (roundoff); bound 5e-6."""
+    lat = P.lattice_as(L.octet(4) if name == "octet" else L.bcc(5, jitter=0.05, radius_range=(0.05, 0.09)), np.float32)
+    g = {}
+    for dtype in (np.float32, np.float64):
+        mm = liblm.MetaMesh(*P.to_device(lat, dtype))
+        gx, gr, _, _ = mm.backward(k, 1.0, 0.5)
+        g[dtype] = np.concatenate([gx.cpu().numpy(), gr.cpu().numpy()[:, None]], 1).astype(np.float64)
+        mm.close()
+    assert np.linalg.norm(g[np.float32] - g[np.float64]) < 5e-6 * np.linalg.norm(g[np.float64])
+
+
+@pytest.mark.parametrize("seed", [2, 5])
+def test_adjoint_of_degenerate_nodes(seed):
+    """FP64 gradients of the area on an irregular lattice (steep sections,
+    sections past a strut's length, seams cut by a plane) against finite
+    differences, at the entries where two step sizes agree to 1e-7 (others
+    sit next to a tangency, where differences do not converge): at least half
+    of them, rows of nodes with cut seams among them.  Not of the volume:
+    such nodes leave the mesh open, and the adjoint's n / 6 per corner is the
+    derivative of a closed mesh's volume."""
+    lat = P.lattice_as(L.irregular(60, seed=seed, r_scale=0.3), np.float64)
+    o = oracle.Oracle(lat)
+    cut = np.array([o.node(n)["flags"] & 32 != 0 for n in range(o.N)])
+    fz = oracle.Frozen(o, 9)
+    d = [fz.fd(h, np.arange(o.N))[0] for h in (1e-4, 5e-5, 2.5e-5)]
+    coarse, ref = (4.0 * d[1] - d[0]) / 3.0, (4.0 * d[2] - d[1]) / 3.0
+    scale = np.maximum(np.abs(ref), 1e-3 * np.median(np.abs(ref).max(1)))
+    sure = np.abs(coarse - ref) < 1e-7 * scale
+    assert sure.mean() > 0.5 and (sure.all(1) & cut).any()
+    mm = liblm.MetaMesh(*P.to_device(lat, np.float64))
+    gx, gr, _, _ = mm.backward(9, 1.0, 0.0)
+    g = np.concatenate([gx.cpu().numpy(), gr.cpu().numpy()[:, None]], 1)
+    assert (np.abs(g - ref) / scale)[sure].max() < 1e-6
+    mm.close()
