@@ -695,7 +695,7 @@ lm_status build_impl(lm_metamesh* mm, cudaStream_t st) {
   mm->flags_or = (uint32_t)hb.stat[1];
   mm->max_loop_entries = (int)hb.stat[2];
   // FP64 fallback contexts of the triangulation kernels
-  mm->scratch_warps = tri_scratch_warps(N, E);
+  mm->scratch_warps = tri_scratch_warps(N);
   {
     const size_t bytes = node64_bytes() * (size_t)mm->scratch_warps;
     cudaError_t se = mm_malloc(mm, (void**)&mm->scratch, bytes, st);
@@ -1080,8 +1080,8 @@ lm_status lm_tri_range(const lm_metamesh* mm, int64_t b, int64_t e, int64_t* h_f
   if (!mm->tri_k) return LM_ERR_STATE;
   int64_t x[2] = {0, mm->tri_total};
   if (b > 0 || e < mm->E + mm->N) {  // the whole range was read back by lm_tri_count
-  if (cudaMemcpy(&x[0], mm->tri_off + b, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return LM_ERR_CUDA;
-  if (cudaMemcpy(&x[1], mm->tri_off + e, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return LM_ERR_CUDA;
+    if (cudaMemcpy(&x[0], mm->tri_off + b, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return LM_ERR_CUDA;
+    if (cudaMemcpy(&x[1], mm->tri_off + e, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return LM_ERR_CUDA;
   }
   if (h_first) *h_first = x[0];
   if (h_count) *h_count = x[1] - x[0];

@@ -311,7 +311,6 @@ struct GenOut {
   uint8_t tangent[2];
   uint8_t nroot;      // 0 or 2 (roots produced, before screening)
   uint8_t unc;        // whole generator uncertain in this precision
-  uint8_t refine;     // decisions certain, but recompute positions in FP64
   uint32_t nflags;    // node flags raised independent of survival
   uint32_t kflags[2]; // node flags raised if the root is kept as a new vertex
   uint64_t umask[2];  // FP32: strut ends whose screening decision was uncertain
@@ -336,7 +335,6 @@ __device__ __forceinline__ void eval_gen_impl(const EndG<U>* E, int d, U R, uint
                                               const GenHint* hint) {
   o.nroot = 0;
   o.unc = 0;
-  o.refine = 0;
   o.nflags = 0;
   int type = gcode & 3, i = (gcode >> 3) & 63, j = (gcode >> 9) & 63, k = (gcode >> 15) & 63;
   uint64_t gmask;

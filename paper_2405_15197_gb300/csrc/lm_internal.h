@@ -181,9 +181,9 @@ cudaError_t metamesh_backward(lm_metamesh* mm, int k, double w_area, double w_vo
 cudaError_t launch_chunk_begin(int64_t* cursor, int64_t stride, int64_t chunk, int64_t i0, int64_t i1, int64_t* range,
                                cudaStream_t st);
 size_t node64_bytes();
-// FP64 contexts of the triangulation kernels for a lattice of N nodes and E
-// struts (the kernels' grids are clamped to them)
-int64_t tri_scratch_warps(int64_t N, int64_t E);
+// FP64 contexts of the triangulation kernels for a lattice of N nodes (the
+// kernels' grids are clamped to them)
+int64_t tri_scratch_warps(int64_t N);
 // device memory of the library: the current device's private pool (see
 // lm_pool_retain); freed with cudaFreeAsync
 cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t st);

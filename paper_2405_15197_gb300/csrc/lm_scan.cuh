@@ -83,17 +83,6 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(const I* in, int64_
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) out[n] = off;
 }
 
-// Workspace (int64 elements) needed by scan_excl for n inputs.
-inline int64_t scan_workspace(int64_t n) {
-  int64_t w = 0;
-  while (n > SCAN_TILE) {
-    int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
-    w += nb + 1;
-    n = nb;
-  }
-  return w + 1;
-}
-
 // out[0..n] = exclusive scan of in[0], in[stride], ...; out[n] = total
 template <typename I>
 cudaError_t scan_excl(const I* in, int64_t stride, int64_t n, int64_t* out, int64_t* ws,

@@ -4,7 +4,7 @@ namespace lm {
 template cudaError_t launch_tri_count<float>(const TriLaunch<float>&, cudaStream_t);
 template cudaError_t launch_tri_emit<float>(const TriLaunch<float>&, cudaStream_t);
 size_t node64_bytes() { return sizeof(Node64); }
-int64_t tri_scratch_warps(int64_t N, int64_t) {
+int64_t tri_scratch_warps(int64_t N) {
   // the hole fans take two per warp of their persistent grid
   const int64_t n = 2 * ((N + 7) / 8 * 8), most = 152 * 64 * 2;
   return n < 16 ? 16 : (n < most ? n : most);
