@@ -64,11 +64,11 @@ WORKLOADS = {
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per triangle of
 # the FP32 stitching launch k_tri_tiles at k = 32 (its FP64 and hole-fan
 # launches take 1.4 % of the emit's time on BCC), measured with ncu on the
-# profiling case of the lattice family (BCC 40^3: 1,727.8 MB over 32.7 M
+# profiling case of the lattice family (BCC 40^3: 1,731.2 MB over 32.7 M
 # triangles of one launch) with the current kernels; the benchmark scales it
 # by the triangles of its own emit (no entry: not measured with the current
 # kernels, reported as null)
-TRAFFIC_PER_TRI_K32 = {"bcc": 52.8}
+TRAFFIC_PER_TRI_K32 = {"bcc": 52.9}
 
 
 METRIC = "meta-mesh struts/s; triangles/s & write GB/s vs HBM peak; adjoint struts/s"

@@ -131,14 +131,18 @@ cudaError_t launch_tri_emit(const TriLaunch<T>& a, cudaStream_t st) {
   // per-tile shared memory fits; otherwise (very fine resolutions) one thread
   // per strut that streams its points
   if (a.item_begin < a.n_struts) {
-    // the FP64 pass (about 1 % of the struts) is bound by the FP64 pipe (1/64
-    // of the FP32 rate) and its steps occupy few lanes: two deferred struts
-    // per warp (16-lane tiles) fill its instructions better than one
+    // the FP64 pass (about 1 % of the struts) is bound by instruction fetch and
+    // by the latency of one strut's steps, which occupy few lanes: two deferred
+    // struts per warp (16-lane tiles) fill its instructions better than one
+    // (octet 24^3, k = 32: 1.10 ms both passes, 1.18 with 32-lane tiles;
+    // irregular 100,000 nodes, k = 16, the other way: 6.50 and 5.63)
     constexpr int TL = 8, TLX = 16;
     const int64_t n = (a.item_end < a.n_struts ? a.item_end : a.n_struts) - a.item_begin;
     TileLayout<T, TL> Lay{a.pmax, a.emax, false, false, a.dmax};
     TileLayout<T, TLX> LayX{a.pmax, a.emax, true, false, a.dmax};
     const size_t smem_cap = 200 * 1024;
+    // (two 8-lane tiles, the least, are half a warp: the kernel's sums run over
+    // the lanes that exist)
     auto tiles_for = [&](size_t bytes, int tl) {
       int t = 128 / tl;
       while (t > 2 && (size_t)t * bytes > smem_cap) t >>= 1;
