@@ -712,7 +712,7 @@ def bench_adjoint(torch, liblm, dev, stream):
     E = int(ends.shape[0])
     return {"struts_per_s": E / (ms / 1e3), "ms": ms, "n_struts": E, "k": 32,
             "workload": "BCC 64^3 cells, node jitter N(0, 0.05), radii U[0.05, 0.09], d(area + volume)/d(xyz, R)",
-            "includes": "objective evaluation + point adjoints + per-node forward-mode pass"}
+            "includes": "objective evaluation + point adjoints + per-node reverse sweep"}
 
 
 # ------------------------------------------------------------ CPU oracle timing
