@@ -439,8 +439,9 @@ long long lm_launch_count(void);
  * above goes back to the driver at the next synchronisation, and all of it
  * when an allocation of the library would not fit otherwise.
  * lm_pool_retain(bytes) changes that limit for the current device (0: nothing
- * is kept, and what is idle now is given back; other allocators, PyTorch's for
- * one, cannot use what the pool keeps).  Returns LM_ERR_CUDA if the pool
+ * is kept, and what is idle now is given back).  What the pool keeps shows as
+ * used, but a cudaMalloc of this process that finds no other room, PyTorch's
+ * for one, gets it; other processes do not.  Returns LM_ERR_CUDA if the pool
  * cannot be made or set.                                                  */
 lm_status lm_pool_retain(uint64_t bytes);
 

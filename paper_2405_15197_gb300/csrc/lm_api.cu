@@ -64,7 +64,8 @@ lm_status st_cuda(cudaError_t e) {
 // with the default pool every synchronisation unmapped what was free, and a
 // build mapped it again (36 allocations of about 10 us on a small part, 27 ms
 // of a 323 ms build of octet 100^3).  What it keeps is given back when
-// an allocation does not fit and by lm_pool_retain(0).
+// an allocation does not fit (the library's, or a cudaMalloc of the process:
+// the driver does that) and by lm_pool_retain(0).
 struct DevPool {
   cudaMemPool_t pool = nullptr;
 };

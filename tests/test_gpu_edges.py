@@ -6,7 +6,8 @@
 * struts whose length, radius or taper leaves the range of the lattice's type;
 * an objective whose sums leave the range of FP32;
 * a device with room for the build but not for the arena beside it;
-* memory that the pool keeps, and gives back on request.
+* memory that the pool keeps, and gives back on request or when PyTorch's
+  allocator has no other.
 """
 import numpy as np
 import pytest
@@ -190,3 +191,21 @@ def test_pool_keeps_and_gives_back():
     liblm.lm_pool_retain(0)
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] > free0 - (64 << 20)
+
+
+def test_records_where_the_pool_holds_the_room():
+    """The records of a build fit on a device whose last room the library's
+    pool keeps idle (the arena and the temporaries of BCC 64^3, about 670 MB):
+    PyTorch's cudaMalloc gets it."""
+    x, e, r = P.to_device(P.lattice_as(L.bcc(64, radius=0.05), np.float32), np.float32)
+    mm = liblm.MetaMesh(x, e, r)
+    size = 50 * mm.tri_count(8)
+    torch.cuda.empty_cache()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - size + (300 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        assert mm.triangulate(8).shape[0] * 50 == size
+        assert liblm.lm_last_error(mm.h) == 0
+    finally:
+        del filler
+        mm.close()
+        torch.cuda.empty_cache()
